@@ -49,7 +49,10 @@ constexpr int RESIDENT_ITERS = 512;
 // Barrier over the grid's blocks, in two halves: what any block wrote before its
 // grid_arrive is visible to every block after its grid_wait; between the two a
 // block does work that needs no other block's.  CLUSTER: the grid is one
-// thread-block cluster, whose hardware barrier does it.  Otherwise sc->bar
+// thread-block cluster, whose hardware barrier does it, in the form that each
+// thread executes for itself: both halves follow branches that a warp need not
+// take as a whole (the sites of a ragged last block, lane 0 of a block sum), and
+// the .aligned form asks for converged warps.  Otherwise sc->bar
 // counts arrivals (0 at the launch) and thread 0, which keeps the next target,
 // waits for it: one release-add that nobody waits for and a polled acquire
 // load.  Bounded: a block that waits too long sets sc->bar_abort, and every
@@ -58,7 +61,7 @@ template <bool CLUSTER>
 __device__ __forceinline__ void grid_arrive(CgScalars *sc, unsigned &target)
 {
     if constexpr (CLUSTER) {
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     } else {
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -71,7 +74,7 @@ template <bool CLUSTER>
 __device__ __forceinline__ bool grid_wait(CgScalars *sc, unsigned target)
 {
     if constexpr (CLUSTER) {
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
         return true;
     } else {
         __shared__ int good;
