@@ -258,7 +258,8 @@ lqcd_status lqcd_dslash(lqcd_field *out, const lqcd_field *U, const lqcd_field *
  *      spinor carried as pairs in Blackwell's packed FP32x2 instructions.
  * Forms 0 and 1 give bitwise the same results; form 2 rounds its products in
  * another order (agreement within FP32 rounding).  The multi-system solver
- * (lqcd_cg_solve_batch, batched chains, solve service) follows the setting.
+ * (lqcd_cg_solve_batch, batched chains, solve service) follows the setting; a
+ * single solve keeps the form and the tuned block size that held at its start.
  * lqcd_dslash_form(form) selects the form (0, 1, 2; a negative value queries)
  * and returns the previous one (process-wide); an unknown form returns -1,
  * leaves the setting unchanged and sets lqcd_last_error. */

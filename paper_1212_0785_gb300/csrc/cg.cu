@@ -647,6 +647,7 @@ lqcd_status CgRun::start_enqueue_impl(cudaStream_t s)
         LQCD_CUDA(cudaMemcpyAsync(w.p64.f->data, w.r64.f->data, b->bytes, cudaMemcpyDeviceToDevice, s));
         P = w.p64.f, R = w.r64.f, T = w.t64a.f, TMP = w.tmpo64.f, XS = x, UU = U;
     }
+    plan = hop_plan(P);
     return LQCD_OK;
 }
 
@@ -702,11 +703,11 @@ lqcd_status CgRun::iterate(cudaStream_t s)
     // follows it, or in its last block; the pause decision and beta from the
     // last block of the CG-update hop (cg_finish)
     PapStep pap;
-    if (hop_takes_pap_step(P->prec)) pap = {sc, partials, hop_partials(P)};
-    LQCD_TRY(dslash_plain(TMP, UU, P, 0, skip, s));
-    LQCD_TRY(dslash_xpay(T, UU, TMP, 0, P, -k2, partials, skip, s, pap.sc ? nullptr : sc));
-    LQCD_TRY(dslash_plain(TMP, UU, T, 1, skip, s, pap));
-    LQCD_TRY(dslash_cg(UU, TMP, 1, T, -k2, XS, R, P, partials, sc, s));
+    if (hop_takes_pap_step(P->prec, plan)) pap = {sc, partials, hop_partials(P, plan)};
+    LQCD_TRY(dslash_plain(TMP, UU, P, 0, skip, s, {}, &plan));
+    LQCD_TRY(dslash_xpay(T, UU, TMP, 0, P, -k2, partials, skip, s, pap.sc ? nullptr : sc, &plan));
+    LQCD_TRY(dslash_plain(TMP, UU, T, 1, skip, s, pap, &plan));
+    LQCD_TRY(dslash_cg(UU, TMP, 1, T, -k2, XS, R, P, partials, sc, s, &plan));
     return launch_p_update(P, R, sc, s);
 }
 

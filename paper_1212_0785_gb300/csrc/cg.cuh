@@ -90,6 +90,7 @@ struct CgRun {
     int Vh = 0;
     lqcd_field *P = nullptr, *R = nullptr, *T = nullptr, *TMP = nullptr, *XS = nullptr;
     const lqcd_field *UU = nullptr;
+    HopPlan plan; // the hopping term's settings when the solve started
     CgScalars *sc = nullptr; // device scalars of this solve
     CgScalars h0{};
     lqcd_cg_info inf{};

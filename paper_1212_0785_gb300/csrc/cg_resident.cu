@@ -464,7 +464,7 @@ lqcd_status CgRun::iterate_resident(cudaStream_t s, bool *launched)
     case LQCD_F64: return launch_resident<LQCD_F64>(*this, s, launched);
     case LQCD_F32: return launch_resident<LQCD_F32>(*this, s, launched);
     case LQCD_F16N:
-        if (kernel_class_timed(K_DSLASH_F16N_PLAIN) || dslash_form_set(-1) != 2) return LQCD_OK;
+        if (kernel_class_timed(K_DSLASH_F16N_PLAIN) || plan.form != 2) return LQCD_OK;
         return launch_resident<LQCD_F16N>(*this, s, launched);
     case LQCD_BF16: return launch_resident<LQCD_BF16>(*this, s, launched);
     default: return LQCD_OK;

@@ -323,10 +323,9 @@ struct ArithOf<PREC_DF> {
 static std::atomic<int> g_form{2};
 
 template <lqcd_prec P, lqcd_prec GP>
-static int use_form(const Geo &)
+static int use_form(const HopPlan &plan)
 {
-    if (P != LQCD_F16N || GP != LQCD_F16N) return 0;
-    return g_form.load(std::memory_order_relaxed);
+    return P == LQCD_F16N && GP == LQCD_F16N ? plan.form : 0;
 }
 
 // launch kernel K in the form chosen by use_form
@@ -372,16 +371,25 @@ static int packed_block(const lqcd_field *in)
     return (b == 64 || b == 128 || b == 256) ? b : DS_BLOCK;
 }
 
+HopPlan hop_plan(const lqcd_field *in)
+{
+    HopPlan plan;
+    if (in->prec != LQCD_F16N) return plan;
+    plan.form = g_form.load(std::memory_order_relaxed);
+    if (plan.form == 2) plan.block = packed_block(in);
+    return plan;
+}
+
 template <lqcd_prec P, lqcd_prec GP = P>
 static void launch_plain(lqcd_field *out, const lqcd_field *U, const lqcd_field *in, int dagger, const int *skip,
-                         cudaStream_t s, PapStep pap = {})
+                         cudaStream_t s, const HopPlan &plan, PapStep pap = {})
 {
     using R = typename ArithOf<P>::type;
     Geo g = make_geo(in->lat);
-    const int st = use_form<P, GP>(g);
+    const int st = use_form<P, GP>(plan);
     if constexpr (P == LQCD_F16N && GP == LQCD_F16N) {
         if (st == 2) {
-            const int bs = packed_block(in);
+            const int bs = plan.block;
             if (dagger)
                 LQCD_LAUNCH_PACKED(bs, pap.sc ? 1 : 0, dslash_plain, (R, P, GP, true),
                                    (spinor_ref<P>(out), spinor_ref<P>(in), gauge_ref<GP>(U), g, out_parity(out), skip,
@@ -415,14 +423,14 @@ static void launch_plain(lqcd_field *out, const lqcd_field *U, const lqcd_field 
 
 template <lqcd_prec P, lqcd_prec GP = P>
 static void launch_xpay(lqcd_field *out, const lqcd_field *U, const lqcd_field *in, int dagger, const lqcd_field *x,
-                        double b, double *partials, const int *skip, cudaStream_t s, CgScalars *fin)
+                        double b, double *partials, const int *skip, cudaStream_t s, CgScalars *fin, const HopPlan &plan)
 {
     using R = typename ArithOf<P>::type;
     Geo g = make_geo(in->lat);
-    const int st = use_form<P, GP>(g);
+    const int st = use_form<P, GP>(plan);
     if constexpr (P == LQCD_F16N && GP == LQCD_F16N) {
         if (st == 2) {
-            const int bs = packed_block(in), nb = nblocks_for(g.Vh, bs);
+            const int bs = plan.block, nb = nblocks_for(g.Vh, bs);
             if (dagger)
                 LQCD_LAUNCH_PACKED(bs, 0, dslash_xpay, (R, P, GP, true),
                                    (spinor_ref<P>(out), spinor_ref<P>(in), gauge_ref<GP>(U), g, out_parity(out),
@@ -463,15 +471,15 @@ static void launch_xpay(lqcd_field *out, const lqcd_field *U, const lqcd_field *
 template <lqcd_prec P, lqcd_prec XP>
 static void launch_cg(const lqcd_field *U, const lqcd_field *in, int dagger, const lqcd_field *t, double b,
                       lqcd_field *xs, lqcd_field *r, const lqcd_field *p, double *partials, CgScalars *sc,
-                      cudaStream_t s)
+                      cudaStream_t s, const HopPlan &plan)
 {
     using R = typename ArithOf<P>::type;
     Geo g = make_geo(in->lat);
     int op = out_parity(t);
-    const int st = use_form<P, P>(g);
+    const int st = use_form<P, P>(plan);
     if constexpr (P == LQCD_F16N) {
         if (st == 2) {
-            const int bs = packed_block(in), nb = nblocks_for(g.Vh, bs);
+            const int bs = plan.block, nb = nblocks_for(g.Vh, bs);
             if (dagger)
                 LQCD_LAUNCH_PACKED(bs, 0, dslash_cg, (R, P, P, true, XP),
                                    (spinor_ref<P>(in), gauge_ref<P>(U), g, op, spinor_ref<P>(t), (R)b,
@@ -519,34 +527,25 @@ int dslash_form_set(int form)
     return g_form.exchange(form);
 }
 
-bool hop_takes_pap_step(lqcd_prec p)
-{
-    return p == LQCD_BF16 || (p == LQCD_F16N && g_form.load(std::memory_order_relaxed) == 2);
-}
-
-int hop_partials(const lqcd_field *in)
-{
-    return nblocks_for(in->Vh, in->prec == LQCD_F16N && hop_takes_pap_step(in->prec) ? packed_block(in) : DS_BLOCK);
-}
-
 lqcd_status dslash_plain(lqcd_field *out, const lqcd_field *U, const lqcd_field *in, int dagger, const int *skip,
-                         cudaStream_t s, PapStep pap)
+                         cudaStream_t s, PapStep pap, const HopPlan *set)
 {
     LQCD_TRY(check_pair(out, U, in));
-    LQCD_REQUIRE(!pap.sc || hop_takes_pap_step(in->prec), "dslash: no CG step beside this hop");
+    const HopPlan plan = set ? *set : hop_plan(in);
+    LQCD_REQUIRE(!pap.sc || hop_takes_pap_step(in->prec, plan), "dslash: no CG step beside this hop");
     double site = 8 * link_bytes(U->prec) + 2 * spinor_site_bytes(in->prec);
     KernelTimer kt(dslash_class(in->prec), s, site * in->Vh);
     KernelTimer kt_plain(in->prec == LQCD_F16N ? K_DSLASH_F16N_PLAIN : K_NCLASS, s, site * in->Vh);
     switch (in->prec) {
-    case LQCD_F64: launch_plain<LQCD_F64>(out, U, in, dagger, skip, s); break;
+    case LQCD_F64: launch_plain<LQCD_F64>(out, U, in, dagger, skip, s, plan); break;
     case LQCD_F32:
         if (U->prec == LQCD_F64)
-            launch_plain<LQCD_F32, LQCD_F64>(out, U, in, dagger, skip, s);
+            launch_plain<LQCD_F32, LQCD_F64>(out, U, in, dagger, skip, s, plan);
         else
-            launch_plain<LQCD_F32>(out, U, in, dagger, skip, s);
+            launch_plain<LQCD_F32>(out, U, in, dagger, skip, s, plan);
         break;
-    case LQCD_F16N: launch_plain<LQCD_F16N>(out, U, in, dagger, skip, s, pap); break;
-    case LQCD_BF16: launch_plain<LQCD_BF16>(out, U, in, dagger, skip, s, pap); break;
+    case LQCD_F16N: launch_plain<LQCD_F16N>(out, U, in, dagger, skip, s, plan, pap); break;
+    case LQCD_BF16: launch_plain<LQCD_BF16>(out, U, in, dagger, skip, s, plan, pap); break;
     default: dslash_df_launch(out, U, in, dagger, nullptr, 0.0, skip, s); break;
     }
     LQCD_LAUNCHED();
@@ -554,22 +553,24 @@ lqcd_status dslash_plain(lqcd_field *out, const lqcd_field *U, const lqcd_field 
 }
 
 lqcd_status dslash_xpay(lqcd_field *out, const lqcd_field *U, const lqcd_field *in, int dagger, const lqcd_field *x,
-                        double b, double *partials, const int *skip, cudaStream_t s, CgScalars *fin)
+                        double b, double *partials, const int *skip, cudaStream_t s, CgScalars *fin,
+                        const HopPlan *set)
 {
     LQCD_TRY(check_pair(out, U, in));
+    const HopPlan plan = set ? *set : hop_plan(in);
     LQCD_REQUIRE(x && x->kind == out->kind && x->prec == out->prec, "dslash_xpay: x must match out");
     double site = 8 * link_bytes(U->prec) + 3 * spinor_site_bytes(in->prec); // + read of x
     KernelTimer kt(dslash_class(in->prec), s, site * in->Vh);
     switch (in->prec) {
-    case LQCD_F64: launch_xpay<LQCD_F64>(out, U, in, dagger, x, b, partials, skip, s, fin); break;
+    case LQCD_F64: launch_xpay<LQCD_F64>(out, U, in, dagger, x, b, partials, skip, s, fin, plan); break;
     case LQCD_F32:
         if (U->prec == LQCD_F64)
-            launch_xpay<LQCD_F32, LQCD_F64>(out, U, in, dagger, x, b, partials, skip, s, fin);
+            launch_xpay<LQCD_F32, LQCD_F64>(out, U, in, dagger, x, b, partials, skip, s, fin, plan);
         else
-            launch_xpay<LQCD_F32>(out, U, in, dagger, x, b, partials, skip, s, fin);
+            launch_xpay<LQCD_F32>(out, U, in, dagger, x, b, partials, skip, s, fin, plan);
         break;
-    case LQCD_F16N: launch_xpay<LQCD_F16N>(out, U, in, dagger, x, b, partials, skip, s, fin); break;
-    case LQCD_BF16: launch_xpay<LQCD_BF16>(out, U, in, dagger, x, b, partials, skip, s, fin); break;
+    case LQCD_F16N: launch_xpay<LQCD_F16N>(out, U, in, dagger, x, b, partials, skip, s, fin, plan); break;
+    case LQCD_BF16: launch_xpay<LQCD_BF16>(out, U, in, dagger, x, b, partials, skip, s, fin, plan); break;
     default:
         LQCD_REQUIRE(partials == nullptr, "float-float hopping term has no norm reduction");
         dslash_df_launch(out, U, in, dagger, x, b, skip, s);
@@ -581,17 +582,18 @@ lqcd_status dslash_xpay(lqcd_field *out, const lqcd_field *U, const lqcd_field *
 
 lqcd_status dslash_cg(const lqcd_field *U, const lqcd_field *in, int dagger, const lqcd_field *t, double b,
                       lqcd_field *xs, lqcd_field *r, const lqcd_field *p, double *partials, CgScalars *sc,
-                      cudaStream_t s)
+                      cudaStream_t s, const HopPlan *set)
 {
+    const HopPlan plan = set ? *set : hop_plan(in);
     // links, input; reads of t, p, r and xs; writes of r and xs (no output of the product)
     double site = 8 * link_bytes(U->prec) + 4 * spinor_site_bytes(in->prec) + spinor_site_bytes(r->prec) +
                   2 * spinor_site_bytes(xs->prec);
     KernelTimer kt(dslash_class(in->prec), s, site * in->Vh);
     switch (in->prec) {
-    case LQCD_F64: launch_cg<LQCD_F64, LQCD_F64>(U, in, dagger, t, b, xs, r, p, partials, sc, s); break;
-    case LQCD_F32: launch_cg<LQCD_F32, LQCD_F32>(U, in, dagger, t, b, xs, r, p, partials, sc, s); break;
-    case LQCD_F16N: launch_cg<LQCD_F16N, LQCD_F32>(U, in, dagger, t, b, xs, r, p, partials, sc, s); break;
-    case LQCD_BF16: launch_cg<LQCD_BF16, LQCD_F32>(U, in, dagger, t, b, xs, r, p, partials, sc, s); break;
+    case LQCD_F64: launch_cg<LQCD_F64, LQCD_F64>(U, in, dagger, t, b, xs, r, p, partials, sc, s, plan); break;
+    case LQCD_F32: launch_cg<LQCD_F32, LQCD_F32>(U, in, dagger, t, b, xs, r, p, partials, sc, s, plan); break;
+    case LQCD_F16N: launch_cg<LQCD_F16N, LQCD_F32>(U, in, dagger, t, b, xs, r, p, partials, sc, s, plan); break;
+    case LQCD_BF16: launch_cg<LQCD_BF16, LQCD_F32>(U, in, dagger, t, b, xs, r, p, partials, sc, s, plan); break;
     }
     LQCD_LAUNCHED();
     return LQCD_OK;

@@ -160,21 +160,40 @@ __device__ __forceinline__ void pap_step(const PapStep &f)
     const double total = block_final_sum<BLOCK>(f.partials, f.n);
     if (threadIdx.x == 0) cg_pap_step(f.sc, total);
 }
+
+// The process-wide settings of the FP16+norm hopping term (dslash_form_set and
+// the autotuner's table), read once for all launches that have to agree: the
+// form decides whether a plain hop takes a PapStep, the block size how many
+// partials a reducing hop stores.  A solve keeps the one it started with, so
+// that a change by another thread meanwhile does not reach it.
+struct HopPlan {
+    int form = 2;
+    int block = DS_BLOCK; // threads per block of the packed FP16+norm kernels
+};
+HopPlan hop_plan(const lqcd_field *in);
 // whether the plain hop of this storage takes a PapStep (the 16-bit packed forms)
-bool hop_takes_pap_step(lqcd_prec p);
+inline bool hop_takes_pap_step(lqcd_prec p, const HopPlan &plan)
+{
+    return p == LQCD_BF16 || (p == LQCD_F16N && plan.form == 2);
+}
 // block partials that a reducing hop on this lattice stores
-int hop_partials(const lqcd_field *in);
+inline int hop_partials(const lqcd_field *in, const HopPlan &plan)
+{
+    return nblocks_for(in->Vh, in->prec == LQCD_F16N && plan.form == 2 ? plan.block : DS_BLOCK);
+}
 
 // out = D_{out<-in} in (dagger: D^dag).  Parities from the field kinds.
-// pap (optional, hop_takes_pap_step): applied beside the hop.
+// pap (optional, hop_takes_pap_step): applied beside the hop.  plan (here and
+// below): NULL takes the settings of the moment.
 lqcd_status dslash_plain(lqcd_field *out, const lqcd_field *U, const lqcd_field *in, int dagger, const int *skip,
-                         cudaStream_t s, PapStep pap = {});
+                         cudaStream_t s, PapStep pap = {}, const HopPlan *plan = nullptr);
 
 // out = x + b D in; if partials != NULL also the per-block partial sums of
 // |out|^2 (dslash_blocks(Vh) of them), and if fin != NULL the last block then
 // sums them and applies the CG pAp step to fin (cg_finish).
 lqcd_status dslash_xpay(lqcd_field *out, const lqcd_field *U, const lqcd_field *in, int dagger, const lqcd_field *x,
-                        double b, double *partials, const int *skip, cudaStream_t s, CgScalars *fin = nullptr);
+                        double b, double *partials, const int *skip, cudaStream_t s, CgScalars *fin = nullptr,
+                        const HopPlan *plan = nullptr);
 
 // CG update fused into the last half of Mhat^dag Mhat:
 //   Ap = t + b D in;  xs += alpha p;  r -= alpha Ap;  partials of |r|^2,
@@ -182,7 +201,7 @@ lqcd_status dslash_xpay(lqcd_field *out, const lqcd_field *U, const lqcd_field *
 // the sloppy precision of in; xs F64 (plain FP64 solve) or F32 (mixed solve).
 lqcd_status dslash_cg(const lqcd_field *U, const lqcd_field *in, int dagger, const lqcd_field *t, double b,
                       lqcd_field *xs, lqcd_field *r, const lqcd_field *p, double *partials, CgScalars *sc,
-                      cudaStream_t s);
+                      cudaStream_t s, const HopPlan *plan = nullptr);
 
 // the FP16+norm hopping-term form: 2 prefetched links with packed FP32x2
 // arithmetic (default), 1 prefetched links, 0 gathered; returns the previous
