@@ -292,6 +292,7 @@ lqcd_status CgWorkspace::ensure_mre(int n, cudaStream_t s)
             return rc;
         }
     }
+    if (mre_tab.bytes < 2 * MRE_MAX * sizeof(float4 *)) LQCD_TRY(mre_tab.alloc(2 * MRE_MAX * sizeof(float4 *), s));
     // each field only if missing, so a call that failed half way can be repeated
     if (!mre_te.f) LQCD_TRY(lqcd_field_alloc(&lat, LQCD_SPINOR_EVEN, LQCD_F32, 0, &mre_te.f));
     if (!mre_to.f) LQCD_TRY(lqcd_field_alloc(&lat, LQCD_SPINOR_ODD, LQCD_F32, 0, &mre_to.f));
@@ -504,7 +505,6 @@ lqcd_status CgRun::mre_refine(cudaStream_t s, double *rr0)
         ptrs[j] = (const float4 *)w.mre_d[j].f->data;
         ptrs[CgWorkspace::MRE_MAX + j] = (const float4 *)w.mre_w[j].f->data;
     }
-    if (w.mre_tab.bytes < sizeof(ptrs)) LQCD_TRY(w.mre_tab.alloc(sizeof(ptrs), s));
     LQCD_CUDA(cudaMemcpyAsync(w.mre_tab.p, ptrs, sizeof(ptrs), cudaMemcpyHostToDevice, s));
     const float4 *const *dtab = (const float4 *const *)w.mre_tab.p;
     const float4 *const *wtab = dtab + CgWorkspace::MRE_MAX;

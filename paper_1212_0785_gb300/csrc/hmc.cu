@@ -839,7 +839,12 @@ static lqcd_status batch_solve(lqcd_batch *B, const lqcd_hmc_params *p, cudaStre
             st->n_solves++;
             continue;
         }
+        // the solver's buffers outlive the batch and its streams: they are made
+        // here, in the order of the caller's stream (those of the guess's
+        // refinement once there are solutions that prepare_guess may pass on)
         LQCD_TRY(st->ws.ensure(st->U->lat, p[i].cg.sloppy, s));
+        if (p[i].chrono >= 2 && p[i].chrono_mre && p[i].cg.sloppy != LQCD_F64 && t.have_guess && t.n_hist >= 2)
+            LQCD_TRY(st->ws.ensure_mre(std::min(p[i].chrono, t.n_hist) - 1, s));
     }
     LQCD_TRY(per_chain(B, s, [&](size_t i, cudaStream_t cst) -> lqcd_status {
         if (reused[i]) return LQCD_OK;
