@@ -311,6 +311,18 @@ typedef struct {
 lqcd_status lqcd_cg_solve(lqcd_field *x, const lqcd_field *U, const lqcd_field *U_sloppy, const lqcd_field *b,
                           double kappa, const lqcd_cg_params *params, lqcd_cg_info *info, void *stream);
 
+/* On a lattice whose thread blocks all run at the same time, lqcd_cg_solve and
+ * the solves of a trajectory make their iterations in one kernel, separated by
+ * barriers over its blocks.  Its limits, for the solves that the calling thread
+ * makes from now on (0: the default):
+ *   iterations  after which a launch returns to the host, which launches the
+ *               next (512); results do not depend on it;
+ *   polls       of a barrier before a block gives up and the solve returns
+ *               LQCD_ETIMEOUT (2^21, about a second);
+ *   blocks      that are taken to run at the same time (what the device holds).
+ * Meant for tests of those paths. */
+lqcd_status lqcd_solver_limits(int iterations, int polls, int blocks);
+
 /* ------------------------------------------------------------ forces and updates */
 
 /* Gauge (staple) force with its traceless anti-Hermitian projection, fused

@@ -41,10 +41,16 @@
 
 namespace lqcd {
 
-// polls of a barrier before a block gives up (about a second), and iterations
-// after which a launch returns to the host in any case
-constexpr int BAR_POLLS = 1 << 21;
-constexpr int RESIDENT_ITERS = 512;
+// iterations after which a launch returns to the host in any case, polls of a
+// barrier before a block gives up (about a second), and the blocks that are
+// taken to run at the same time (0: what the device says), of the solves that
+// the calling thread makes (lqcd_solver_limits)
+struct ResidentLimits {
+    int iters = 512;
+    int polls = 1 << 21;
+    int blocks = 0;
+};
+static thread_local ResidentLimits t_limits;
 
 // Barrier over the grid's blocks, in two halves: what any block wrote before its
 // grid_arrive is visible to every block after its grid_wait; between the two a
@@ -71,7 +77,7 @@ __device__ __forceinline__ void grid_arrive(CgScalars *sc, unsigned &target)
     }
 }
 template <bool CLUSTER>
-__device__ __forceinline__ bool grid_wait(CgScalars *sc, unsigned target)
+__device__ __forceinline__ bool grid_wait(CgScalars *sc, unsigned target, int polls)
 {
     if constexpr (CLUSTER) {
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
@@ -84,8 +90,8 @@ __device__ __forceinline__ bool grid_wait(CgScalars *sc, unsigned target)
                 unsigned v;
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&sc->bar) : "memory");
                 if (v >= target) break;
-                if (k >= BAR_POLLS) atomicExch(&sc->bar_abort, 1u);
-                if ((k & 63) == 63 || k >= BAR_POLLS) {
+                if (k >= polls) atomicExch(&sc->bar_abort, 1u);
+                if ((k & 63) == 63 || k >= polls) {
                     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&sc->bar_abort) : "memory");
                     if (v) {
                         ok = 0;
@@ -100,10 +106,10 @@ __device__ __forceinline__ bool grid_wait(CgScalars *sc, unsigned target)
     }
 }
 template <bool CLUSTER>
-__device__ __forceinline__ bool grid_barrier(CgScalars *sc, unsigned &target)
+__device__ __forceinline__ bool grid_barrier(CgScalars *sc, unsigned &target, int polls)
 {
     grid_arrive<CLUSTER>(sc, target);
-    return grid_wait<CLUSTER>(sc, target);
+    return grid_wait<CLUSTER>(sc, target, polls);
 }
 
 // blocks per SM the register budget is cut for: they set the largest lattice
@@ -195,7 +201,7 @@ __device__ __forceinline__ Sp<R> resident_site(ResidentHops<SP> &sh, const Spino
 template <lqcd_prec SP, bool CLUSTER>
 __global__ void __launch_bounds__(DS_BLOCK, RESIDENT_PER_SM)
     cg_resident_kernel(SpinorRef<SP> p, SpinorRef<SP> r, SpinorRef<SP> t, SpinorRef<SP> tmp, SpinorRef<LQCD_F32> xs,
-                       GaugeRef<SP> U, Geo g, float b, double *partials, int nb, CgScalars *sc)
+                       GaugeRef<SP> U, Geo g, float b, double *partials, int nb, CgScalars *sc, ResidentLimits lim)
 {
     using R = float;
     constexpr bool PACKED = SP == LQCD_F16N || SP == LQCD_BF16;
@@ -213,7 +219,7 @@ __global__ void __launch_bounds__(DS_BLOCK, RESIDENT_PER_SM)
             resident_neighbours<SP>(hops, g, cb);
             resident_links<SP>(hops, U, cb, 0);
         }
-    for (int it = 0; it < RESIDENT_ITERS; it++) {
+    for (int it = 0; it < lim.iters; it++) {
         // tmp = D p;  t = p + b D tmp, |t|^2;  tmp = D^dag t;  A p = t + b D^dag tmp, r -= alpha A p, |r|^2, x += alpha p
 #pragma unroll 1
         for (int ph = 0; ph < 4; ph++) {
@@ -265,7 +271,7 @@ __global__ void __launch_bounds__(DS_BLOCK, RESIDENT_PER_SM)
                     }
                 xs.store(cb, xv);
             }
-            if (!(ok = grid_wait<CLUSTER>(sc, target))) break;
+            if (!(ok = grid_wait<CLUSTER>(sc, target, lim.polls))) break;
             if (ph == 3) resident_scalars<DS_BLOCK>(s, partials + gridDim.x, nb, true);
             if (ph >= 2 && s.pause) break;
         }
@@ -280,7 +286,7 @@ __global__ void __launch_bounds__(DS_BLOCK, RESIDENT_PER_SM)
                 for (int k = 0; k < 3; k++) pv.c[a][k] = rv.c[a][k] + beta * pv.c[a][k];
             p.store(cb, pv);
         }
-        if (!(ok = grid_barrier<CLUSTER>(sc, target))) break;
+        if (!(ok = grid_barrier<CLUSTER>(sc, target, lim.polls))) break;
     }
     if constexpr (PACKED) cp_async_wait<0>();
     if (blockIdx.x == 0 && threadIdx.x == 0) resident_result(sc, s, ok);
@@ -292,7 +298,7 @@ template <bool CLUSTER>
 __global__ void __launch_bounds__(QUAD_BLOCK, RESIDENT_PER_SM)
     cg_resident_f64_kernel(SpinorRef<LQCD_F64> p, SpinorRef<LQCD_F64> r, SpinorRef<LQCD_F64> t, SpinorRef<LQCD_F64> tmp,
                            SpinorRef<LQCD_F64> xs, GaugeRef<LQCD_F64> U, Geo g, double b, double *partials, int nb,
-                           CgScalars *sc)
+                           CgScalars *sc, ResidentLimits lim)
 {
     __shared__ QuadF64 sh;
     __shared__ CgScalars s;
@@ -303,7 +309,7 @@ __global__ void __launch_bounds__(QUAD_BLOCK, RESIDENT_PER_SM)
     const bool live = cb < g.Vh;
     unsigned target = 0;
     bool ok = true;
-    for (int it = 0; it < RESIDENT_ITERS; it++) {
+    for (int it = 0; it < lim.iters; it++) {
 #pragma unroll 1
         for (int ph = 0; ph < 4; ph++) {
             const bool odd = ph & 1;
@@ -331,13 +337,13 @@ __global__ void __launch_bounds__(QUAD_BLOCK, RESIDENT_PER_SM)
                 resident_scalars<QUAD_BLOCK>(s, partials, nb, false);
             else if (ph == 3 && live)
                 store_row(xs, cb, row_xpay(load_row(xs, cb), s.alpha, load_row(p, cb)));
-            if (!(ok = grid_wait<CLUSTER>(sc, target))) break;
+            if (!(ok = grid_wait<CLUSTER>(sc, target, lim.polls))) break;
             if (ph == 3) resident_scalars<QUAD_BLOCK>(s, partials + gridDim.x, nb, true);
             if (ph >= 2 && s.pause) break;
         }
         if (!ok || s.pause) break;
         if (live) store_row(p, cb, row_xpay(load_row(r, cb), s.beta, load_row(p, cb)));
-        if (!(ok = grid_barrier<CLUSTER>(sc, target))) break;
+        if (!(ok = grid_barrier<CLUSTER>(sc, target, lim.polls))) break;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) resident_result(sc, s, ok);
 }
@@ -429,7 +435,7 @@ static lqcd_status launch_resident(const CgRun &run, cudaStream_t s, bool *launc
     int nb = nblocks_for(run.Vh, Resident<SP>::SITES);
     const ResidentCapacity cap = resident_capacity<SP>();
     const bool cluster = cap.cluster16 && nb <= CLUSTER_MAX;
-    if (!cluster && nb > cap.blocks) return LQCD_OK;
+    if (!cluster && nb > (t_limits.blocks ? t_limits.blocks : cap.blocks)) return LQCD_OK;
     if (2 * (size_t)std::max(nb, CLUSTER_MAX) * sizeof(double) > run.ws->partials.bytes) return LQCD_OK;
     SpinorRef<SP> p = spinor_ref<SP>(run.P), r = spinor_ref<SP>(run.R), t = spinor_ref<SP>(run.T),
                   tmp = spinor_ref<SP>(run.TMP);
@@ -439,7 +445,8 @@ static lqcd_status launch_resident(const CgRun &run, cudaStream_t s, bool *launc
     R b = (R)(-run.k2);
     double *partials = (double *)run.ws->partials.p;
     CgScalars *sc = run.sc;
-    void *args[] = {&p, &r, &t, &tmp, &xs, &U, &g, &b, &partials, &nb, &sc};
+    ResidentLimits lim = t_limits;
+    void *args[] = {&p, &r, &t, &tmp, &xs, &U, &g, &b, &partials, &nb, &sc, &lim};
     if (cluster) {
         cudaLaunchAttribute attr;
         const cudaLaunchConfig_t cfg = cluster_config(nb, BLOCK, &attr, s);
@@ -472,3 +479,14 @@ lqcd_status CgRun::iterate_resident(cudaStream_t s, bool *launched)
 }
 
 } // namespace lqcd
+
+extern "C" lqcd_status lqcd_solver_limits(int iterations, int polls, int blocks)
+{
+    using namespace lqcd;
+    LQCD_REQUIRE(iterations >= 0 && polls >= 0 && blocks >= 0, "solver_limits: a limit is negative");
+    const ResidentLimits dflt;
+    t_limits.iters = iterations ? iterations : dflt.iters;
+    t_limits.polls = polls ? polls : dflt.polls;
+    t_limits.blocks = blocks;
+    return LQCD_OK;
+}

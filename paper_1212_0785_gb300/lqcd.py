@@ -131,6 +131,7 @@ _SIGS = {
     "lqcd_autotune_clear": (_i, []),
     "lqcd_mhat": (_i, [_vp, _vp, _vp, _d, _i, _vp]),
     "lqcd_cg_solve": (_i, [_vp, _vp, _vp, _vp, _d, ctypes.POINTER(CgParams), ctypes.POINTER(CgInfo), _vp]),
+    "lqcd_solver_limits": (_i, [_i, _i, _i]),
     "lqcd_gauge_force": (_i, [_vp, _vp, _d, _d, _vp]),
     "lqcd_gauge_force_ex": (_i, [_vp, _vp, _d, _d, _i, _vp]),
     "lqcd_fermion_force": (_i, [_vp, _vp, _vp, _d, _d, _vp]),
@@ -457,6 +458,11 @@ def cg_solve(x: Field, U: Field, b: Field, kappa, params: CgParams | None = None
     if check and rc not in (OK, ENOCONV):
         _check(rc, "cg_solve")
     return rc, info
+
+
+def solver_limits(iterations=0, polls=0, blocks=0):
+    """limits of the one-launch solver for this thread's solves; 0: the default"""
+    _check(lib().lqcd_solver_limits(int(iterations), int(polls), int(blocks)), "solver_limits")
 
 
 def gauge_force(P: Field, U: Field, beta, coeff, arith=None, stream=None):
