@@ -91,6 +91,7 @@ struct CgRun {
     lqcd_field *P = nullptr, *R = nullptr, *T = nullptr, *TMP = nullptr, *XS = nullptr;
     const lqcd_field *UU = nullptr;
     HopPlan plan; // the hopping term's settings when the solve started
+    bool resident_refused = false; // the runtime refused the resident kernel's launch
     CgScalars *sc = nullptr; // device scalars of this solve
     CgScalars h0{};
     lqcd_cg_info inf{};

@@ -427,7 +427,7 @@ static ResidentCapacity resident_capacity()
 }
 
 template <lqcd_prec SP>
-static lqcd_status launch_resident(const CgRun &run, cudaStream_t s, bool *launched)
+static lqcd_status launch_resident(CgRun &run, cudaStream_t s, bool *launched)
 {
     using R = typename Resident<SP>::R;
     constexpr lqcd_prec XP = Resident<SP>::XP;
@@ -447,13 +447,22 @@ static lqcd_status launch_resident(const CgRun &run, cudaStream_t s, bool *launc
     CgScalars *sc = run.sc;
     ResidentLimits lim = t_limits;
     void *args[] = {&p, &r, &t, &tmp, &xs, &U, &g, &b, &partials, &nb, &sc, &lim};
+    cudaError_t refused;
     if (cluster) {
         cudaLaunchAttribute attr;
         const cudaLaunchConfig_t cfg = cluster_config(nb, BLOCK, &attr, s);
-        LQCD_CUDA(cudaLaunchKernelExC(&cfg, Resident<SP>::kernel(true), args));
+        refused = cudaLaunchKernelExC(&cfg, Resident<SP>::kernel(true), args);
     } else {
         LQCD_CUDA(cudaMemsetAsync(&sc->bar, 0, 2 * sizeof(unsigned int), s)); // bar and bar_abort
-        LQCD_CUDA(cudaLaunchCooperativeKernel(Resident<SP>::kernel(false), dim3(nb), dim3(BLOCK), args, 0, s));
+        refused = cudaLaunchCooperativeKernel(Resident<SP>::kernel(false), dim3(nb), dim3(BLOCK), args, 0, s);
+    }
+    // A launch that the runtime refuses (the process may have fewer SMs than the
+    // device's attributes say) leaves the solve as it was: it goes on kernel by
+    // kernel.  An error of the context itself comes back from those launches.
+    if (refused != cudaSuccess) {
+        cudaGetLastError();
+        run.resident_refused = true;
+        return LQCD_OK;
     }
     LQCD_LAUNCHED();
     *launched = true;
@@ -463,6 +472,7 @@ static lqcd_status launch_resident(const CgRun &run, cudaStream_t s, bool *launc
 lqcd_status CgRun::iterate_resident(cudaStream_t s, bool *launched)
 {
     *launched = false;
+    if (resident_refused) return LQCD_OK;
     const lqcd_prec sp = mixed ? prm.sloppy : LQCD_F64;
     // timed hopping-term classes count and time single launches; the resident
     // kernel has the default form of the FP16+norm hopping term

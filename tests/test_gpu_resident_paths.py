@@ -99,6 +99,17 @@ def test_barrier_that_gives_up(prec):
     assert p.solve()[0] == ref
 
 
+@pytest.mark.parametrize("prec,dims", BY_KERNEL)
+def test_refused_launch_goes_kernel_by_kernel(prec, dims):
+    """a grid that the device does not hold at once (or a process with a part of
+    its SMs does not): the runtime refuses the cooperative launch"""
+    p = Problem(dims, prec)
+    ref, n_ref = p.solve()
+    lqcd.solver_limits(blocks=1 << 20)
+    got, n = p.solve()
+    assert got == ref and n == n_ref
+
+
 def test_limits_are_checked():
     for bad in ((-1, 0, 0), (0, -1, 0), (0, 0, -1)):
         with pytest.raises(lqcd.LqcdError):
