@@ -354,20 +354,10 @@ static int use_form(const HopPlan &plan)
     } while (0)
 
 // threads per block of the packed FP16+norm kernels on this lattice: the
-// calling thread's override while the autotuner times a candidate, else the
 // autotuner's choice, else DS_BLOCK
-static thread_local int t_packed_block = 0;
-
-int dslash_packed_block_override(int bs)
-{
-    const int prev = t_packed_block;
-    t_packed_block = bs;
-    return prev;
-}
-
 static int packed_block(const lqcd_field *in)
 {
-    const int b = t_packed_block ? t_packed_block : tuned_block(TK_HOP_F16N, in->lat, DS_BLOCK);
+    const int b = tuned_block(TK_HOP_F16N, in->lat, DS_BLOCK);
     return (b == 64 || b == 128 || b == 256) ? b : DS_BLOCK;
 }
 
@@ -516,7 +506,6 @@ static void launch_cg(const lqcd_field *U, const lqcd_field *in, int dagger, con
     }
 }
 
-// the packed plain hop with bs threads per block, for the autotuner
 int dslash_form_set(int form)
 {
     if (form < 0) return g_form.load();
