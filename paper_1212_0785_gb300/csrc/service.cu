@@ -113,8 +113,11 @@ struct SvcGauge {
     lqcd_field *U = nullptr; // borrowed FP64 links
     FieldPtr Us, Udf;         // sloppy copy and float-float copy shared by every solve on it
     // sets of transient float-float fields shared by its solves: the solves of
-    // one set form their accurate residuals one after another
+    // one set form their accurate residuals one after another.  One is needed;
+    // the others are made where memory allows (grow_sets) and given back where
+    // an admission finds too little (drop_sets)
     std::vector<std::unique_ptr<CgWorkspace>> shared;
+    bool one_set = false; // the others were given back
     // set-up (FP64, zero outside the few sites a set-up writes, cleared after
     // each use) and check (float-float) temporaries, used one solve at a time
     FieldPtr bo, bp, to, src, bo_df, xo_df, mxe_df;
@@ -202,21 +205,40 @@ static size_t rhs_bytes(const lqcd_lattice &lat, lqcd_prec sloppy)
     return ws_bytes(lat, sloppy) + (size_t)make_geo(lat).Vh * 2 * 192;
 }
 
+static lqcd_status add_set(lqcd_service *S, SvcGauge &g)
+{
+    std::unique_ptr<CgWorkspace> t(new CgWorkspace());
+    t->temps_only = true;
+    LQCD_TRY(t->ensure(g.U->lat, S->prm.cg.sloppy, S->stream));
+    g.shared.push_back(std::move(t));
+    return LQCD_OK;
+}
+
+static void count_fixed(lqcd_service *S, SvcGauge &g)
+{
+    size_t fixed = g.part.bytes + g.scal.bytes;
+    for (const auto &t : g.shared) fixed += t->bytes();
+    for (const FieldPtr *f : {&g.Us, &g.Udf, &g.bo, &g.bp, &g.to, &g.src, &g.bo_df, &g.xo_df, &g.mxe_df})
+        fixed += f->f->bytes + f->f->norm_bytes;
+    std::lock_guard<std::mutex> lk(S->mu);
+    g.fixed_bytes = fixed;
+}
+
 static lqcd_status gauge_setup(lqcd_service *S, SvcGauge &g)
 {
     if (g.ready) return LQCD_OK;
     cudaStream_t s = S->stream;
     const lqcd_lattice &lat = g.U->lat;
+    // a set-up that failed half way starts over
+    for (FieldPtr *f : {&g.Us, &g.Udf, &g.bo, &g.bp, &g.to, &g.src, &g.bo_df, &g.xo_df, &g.mxe_df}) {
+        if (f->f) lqcd_field_free(f->f);
+        f->f = nullptr;
+    }
     LQCD_TRY(lqcd_field_alloc(&lat, LQCD_GAUGE, S->prm.cg.sloppy, 12, &g.Us.f));
     LQCD_TRY(lqcd_field_copy(g.Us.f, g.U, s));
     LQCD_TRY(field_alloc_df(&lat, LQCD_GAUGE, &g.Udf.f));
     LQCD_TRY(split_links(g.Udf.f, g.U, s));
-    g.shared.resize(temporary_sets(make_geo(lat).Vh));
-    for (auto &t : g.shared) {
-        if (!t) t.reset(new CgWorkspace());
-        t->temps_only = true;
-        LQCD_TRY(t->ensure(lat, S->prm.cg.sloppy, s));
-    }
+    if (g.shared.empty()) LQCD_TRY(add_set(S, g));
     LQCD_TRY(lqcd_field_alloc(&lat, LQCD_SPINOR_ODD, LQCD_F64, 0, &g.bo.f));
     LQCD_TRY(lqcd_field_alloc(&lat, LQCD_SPINOR_EVEN, LQCD_F64, 0, &g.bp.f));
     LQCD_TRY(lqcd_field_alloc(&lat, LQCD_SPINOR_ODD, LQCD_F64, 0, &g.to.f));
@@ -228,16 +250,44 @@ static lqcd_status gauge_setup(lqcd_service *S, SvcGauge &g)
         LQCD_CUDA(cudaMemsetAsync(f->data, 0, f->bytes, s));
     LQCD_TRY(g.part.alloc(sizeof(double) * (nblocks_for(make_geo(lat).Vh, 256) + 1), s));
     LQCD_TRY(g.scal.alloc(sizeof(double) * 4, s));
-    size_t fixed = g.part.bytes + g.scal.bytes;
-    for (const auto &t : g.shared) fixed += t->bytes();
-    for (const FieldPtr *f : {&g.Us, &g.Udf, &g.bo, &g.bp, &g.to, &g.src, &g.bo_df, &g.xo_df, &g.mxe_df})
-        fixed += f->f->bytes + f->f->norm_bytes;
-    {
-        std::lock_guard<std::mutex> lk(S->mu);
-        g.fixed_bytes = fixed;
-    }
+    count_fixed(S, g);
     g.ready = true;
     return LQCD_OK;
+}
+
+// further sets, beside the right-hand sides of an admitted request and only
+// while there is memory for them; where it ends, one is given back, which is
+// many times the room that the solver's tables take (3 bytes per even site and
+// right-hand side against a set's 576 per even site)
+static void grow_sets(lqcd_service *S, SvcGauge &g)
+{
+    const size_t want = g.one_set ? 1 : temporary_sets(make_geo(g.U->lat).Vh);
+    if (g.shared.size() >= want) return;
+    while (g.shared.size() < want)
+        if (add_set(S, g) != LQCD_OK) {
+            if (g.shared.size() > 1) g.shared.pop_back();
+            break;
+        }
+    count_fixed(S, g);
+}
+
+// all gauge fields back to one set, to which their running solves turn (the
+// sets hold nothing between the solver's steps); returns whether any was freed
+static bool drop_sets(lqcd_service *S)
+{
+    bool any = false;
+    for (auto &g : S->gauges) {
+        g->one_set = true;
+        if (g->shared.size() < 2) continue;
+        any = true;
+        for (SvcRequest *r : S->running)
+            if (S->gauges[r->req.gauge] == g)
+                for (auto &h : r->rhs)
+                    if (h->ws) h->ws->tmp_from = g->shared[0].get();
+        g->shared.resize(1);
+        count_fixed(S, *g);
+    }
+    return any;
 }
 
 // the site lists of a request's source (host; periodic neighbours)
@@ -336,9 +386,9 @@ static lqcd_status rhs_start(lqcd_service *S, SvcGauge &g, SvcRequest &r, SvcRhs
     return LQCD_OK;
 }
 
-static lqcd_status admit(lqcd_service *S, SvcRequest &r)
+// the allocations of an admission, and everything it enqueues
+static lqcd_status admit_enqueue(lqcd_service *S, SvcRequest &r, SvcGauge &g)
 {
-    SvcGauge &g = *S->gauges[r.req.gauge];
     LQCD_TRY(gauge_setup(S, g));
     const lqcd_lattice &lat = g.U->lat;
     LQCD_TRY(source_sites(r, lat, S->stream));
@@ -355,15 +405,31 @@ static lqcd_status admit(lqcd_service *S, SvcRequest &r)
             h->ws.reset(new CgWorkspace());
         }
         h->ws->udf_ext = g.Udf.f;
-        h->ws->tmp_from = g.shared[k % g.shared.size()].get();
+        h->ws->tmp_from = g.shared[0].get();
         LQCD_TRY(h->ws->ensure(lat, S->prm.cg.sloppy, S->stream));
         LQCD_TRY(lqcd_field_alloc(&lat, LQCD_SPINOR_EVEN, LQCD_F64, 0, &h->y.f));
         LQCD_TRY(lqcd_field_alloc(&lat, LQCD_SPINOR_ODD, LQCD_F64, 0, &h->xo.f));
         LQCD_TRY(rhs_start(S, g, r, *h, false));
         r.rhs.push_back(std::move(h));
     }
+    return LQCD_OK;
+}
+
+static lqcd_status admit(lqcd_service *S, SvcRequest &r)
+{
+    SvcGauge &g = *S->gauges[r.req.gauge];
+    lqcd_status rc = admit_enqueue(S, r, g);
+    if (rc == LQCD_ENOMEM && drop_sets(S)) {
+        r.rhs.clear();
+        rc = admit_enqueue(S, r, g);
+    }
+    LQCD_TRY(rc);
+    grow_sets(S, g);
     std::vector<CgRun *> runs;
-    for (auto &h : r.rhs) runs.push_back(&h->run);
+    for (size_t k = 0; k < r.rhs.size(); k++) {
+        r.rhs[k]->ws->tmp_from = g.shared[k % g.shared.size()].get();
+        runs.push_back(&r.rhs[k]->run);
+    }
     LQCD_TRY(S->bs.read_starts(runs, S->stream));
     for (size_t k = 0; k < runs.size(); k++) {
         if (!runs[k]->done) runs[k]->start_finish(S->bs.start_of(k), S->stream);
