@@ -114,10 +114,19 @@ __device__ __forceinline__ void gauge_force_link(MomRef &P, const GaugeRef<GP> &
             m3_scale(up, w);
             m3_scale(lo, w);
         }
-        m3_acc(A, up);
-        m3_acc(A, lo);
+        // FP64: the six staples in pairs, whose sums round at a smaller size, and
+        // the last product split: rms error on 8^4 1.806e-16 against 1.865e-16 as
+        // chains and 1.844e-16 with v + a * b throughout; 1353 against 1336 us on
+        // 16^3x32, bound by the FP64 pipe
+        if constexpr (sizeof(R) == 8) {
+            m3_acc(up, lo);
+            m3_acc(A, up);
+        } else {
+            m3_acc(A, up);
+            m3_acc(A, lo);
+        }
     }
-    M3<R> W = m3_mul(U.template load<R>(mu, par, cb), A);
+    M3<R> W = m3_mul_split(U.template load<R>(mu, par, cb), A);
     R gl[8];
     im_tr_lambda(W, gl);
 #pragma unroll
