@@ -117,7 +117,7 @@ __device__ __forceinline__ void link_update_one(const GaugeRef<LQCD_F64> &U, con
         double p[8];
         for (int a = 0; a < 8; a++) p[a] = P.d[P.idx(mu, par, a, cb)];
         M3<double> E = expi_cayley_hamilton(herm_from_coeffs(p, c));
-        nu = m3_mul(E, U.load<double>(mu, par, cb));
+        nu = m3_mul_split(E, U.load<double>(mu, par, cb));
         if (Udf.d) Udf.store(mu, par, cb, nu);
         for (int i = 0; i < 2; i++)
             for (int j = 0; j < 3; j++) nf.e[i][j] = cx<float>((float)nu.e[i][j].re, (float)nu.e[i][j].im);

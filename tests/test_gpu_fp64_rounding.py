@@ -102,3 +102,27 @@ def test_gauge_force(inputs):
         ref[:, mu, 2] = w[:, 0, 0].imag - w[:, 1, 1].imag
         ref[:, mu, 7] = (w[:, 0, 0].imag + w[:, 1, 1].imag - 2 * w[:, 2, 2].imag) / np.sqrt(L(3))
     check("gauge_force", rms(P.download() + ref, ref))
+
+
+@pytest.mark.parametrize("c", [0.02, 0.1, 0.4, 0.7, 1.0, 4.0])
+def test_link_update(inputs, c):
+    U, _, P = inputs
+    G = lqcd.gauge_field(DIMS).upload(U)
+    lqcd.link_update(G, lqcd.momentum_field(DIMS).upload(P), c)
+    n, p = 512, P[:512].astype(L) * (L(c) / 2)
+    h = np.zeros((n, 4, 3, 3), C)
+    for a, (i, j) in ((0, (0, 1)), (3, (0, 2)), (5, (1, 2))):
+        h[..., i, j], h[..., j, i] = p[..., a] - 1j * p[..., a + 1], p[..., a] + 1j * p[..., a + 1]
+    d = p[..., 7] / np.sqrt(L(3))
+    h[..., 0, 0], h[..., 1, 1], h[..., 2, 2] = p[..., 2] + d, -p[..., 2] + d, -2 * d
+    halvings = 0
+    while 3 * np.abs(h).max() > 0.25 * 2 ** halvings:
+        halvings += 1
+    x, eye = h * (C(1j) / 2 ** halvings), np.eye(3, dtype=C)
+    e = eye + x / 16
+    for k in range(15, 0, -1):  # Taylor series, remainder (1/4)^17 / 17!
+        e = eye + mm(x, e) / k
+    for _ in range(halvings):
+        e = mm(e, e)
+    ref = mm(e, U[:n].astype(C))
+    check(c, rms(G.download()[:n] - ref, ref))
