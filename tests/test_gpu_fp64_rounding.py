@@ -126,3 +126,21 @@ def test_link_update(inputs, c):
         e = mm(e, e)
     ref = mm(e, U[:n].astype(C))
     check(c, rms(G.download()[:n] - ref, ref))
+
+
+def test_reunitarize(inputs):
+    U = inputs[0].copy()
+    U[..., :2, :] = U[..., :2, :].real.astype(np.float16) + 1j * U[..., :2, :].imag.astype(np.float16)
+    G = lqcd.gauge_field(DIMS).upload(U)
+    lqcd.reunitarize(G)
+
+    def norm(a):
+        return np.sqrt((a.real ** 2 + a.imag ** 2).sum(-1, keepdims=True))
+
+    r0, r1 = U[..., 0, :].astype(C), U[..., 1, :].astype(C)
+    r0 = r0 / norm(r0)
+    r1 = r1 - (np.conj(r0) * r1).sum(-1, keepdims=True) * r0
+    r1 = r1 / norm(r1)
+    out = G.download()
+    check("row1", rms(out[..., 1, :] - r1))
+    check("row2", rms(out[..., 2, :] - np.conj(np.cross(r0, r1))))
