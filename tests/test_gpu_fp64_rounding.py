@@ -144,3 +144,20 @@ def test_reunitarize(inputs):
     out = G.download()
     check("row1", rms(out[..., 1, :] - r1))
     check("row2", rms(out[..., 2, :] - np.conj(np.cross(r0, r1))))
+
+
+def test_plaquette():
+    """over links of many 2^4 lattices, whose sums are short enough to show it"""
+    dims, n, v = (2, 2, 2, 2), 2000, 16
+    r = np.random.default_rng(7)
+    got, U = [], []
+    for _ in range(n):
+        U.append(rand_su3(r, v * 4).reshape(v, 4, 3, 3))
+        got.append(lqcd.plaquette(lqcd.gauge_field(dims).upload(U[-1])))
+    u, s = np.array(U).astype(C), np.zeros(n, L)
+    ahead = [np.roll(u.reshape(n, 2, 2, 2, 2, 4, 3, 3), -1, axis=4 - mu).reshape(u.shape) for mu in range(4)]
+    for mu in range(4):
+        for nu in range(mu + 1, 4):
+            a, b = mm(u[:, :, mu], ahead[mu][:, :, nu]), mm(u[:, :, nu], ahead[nu][:, :, mu])
+            s += (a.real * b.real + a.imag * b.imag).sum(axis=(1, 2, 3)) / 3
+    check("plaquette", rms(np.array(got).astype(L) * 6 * v - s))
