@@ -123,7 +123,7 @@ __device__ __forceinline__ void hop_dir_df(DfAcc (&ar)[4], DfAcc (&ai)[4], const
 {
     const bool antip = (MU == 3) && g.t_bc < 0;
     { // forward: row a of U_mu(x)
-        DfAcc r0, i0, r1, i1;
+        DfDot r0, i0, r1, i1;
 #pragma unroll
         for (int b = 0; b < 3; b++) {
             float4 w = ldg(U.d + U.idx(MU, out_par, a * 3 + b, cb));
@@ -140,10 +140,10 @@ __device__ __forceinline__ void hop_dir_df(DfAcc (&ar)[4], DfAcc (&ai)[4], const
                 r1.add_prod(ur, h1.re);
                 i1.add_prod(ur, h1.im);
             }
-            r0.sub_prod(ui, h0.im);
-            i0.add_prod(ui, h0.re);
-            r1.sub_prod(ui, h1.im);
-            i1.add_prod(ui, h1.re);
+            r0.sub_prod<1>(ui, h0.im);
+            i0.add_prod<1>(ui, h0.re);
+            r1.sub_prod<1>(ui, h1.im);
+            i1.add_prod<1>(ui, h1.re);
         }
         Cx<Df> v0{r0.raw(), i0.raw()}, v1{r1.raw(), i1.raw()};
         if (antip && wrap_f) {
@@ -153,7 +153,7 @@ __device__ __forceinline__ void hop_dir_df(DfAcc (&ar)[4], DfAcc (&ai)[4], const
         acc_hop<MU, FS, MU == 0>(ar, ai, v0, v1);
     }
     { // backward: column a of U_mu(x - mu), conjugated
-        DfAcc r0, i0, r1, i1;
+        DfDot r0, i0, r1, i1;
 #pragma unroll
         for (int b = 0; b < 3; b++) {
             float4 w = ldg(U.d + U.idx(MU, 1 - out_par, b * 3 + a, nbk));
@@ -170,10 +170,10 @@ __device__ __forceinline__ void hop_dir_df(DfAcc (&ar)[4], DfAcc (&ai)[4], const
                 r1.add_prod(ur, h1.re);
                 i1.add_prod(ur, h1.im);
             }
-            r0.add_prod(ui, h0.im);
-            i0.sub_prod(ui, h0.re);
-            r1.add_prod(ui, h1.im);
-            i1.sub_prod(ui, h1.re);
+            r0.add_prod<1>(ui, h0.im);
+            i0.sub_prod<1>(ui, h0.re);
+            r1.add_prod<1>(ui, h1.im);
+            i1.sub_prod<1>(ui, h1.re);
         }
         Cx<Df> v0{r0.raw(), i0.raw()}, v1{r1.raw(), i1.raw()};
         if (antip && wrap_b) {

@@ -842,17 +842,17 @@ __device__ __forceinline__ double plaq_plane(const GaugeRef<LQCD_F64> &U, int mu
 // row (r[0], r[1], r[2]) times column j of u
 __device__ __forceinline__ Cx<Df> df_row_times(const Cx<Df> (&r)[3], const M3<Df> &u, int j)
 {
-    DfAcc re, im;
+    DfDot re, im;
     re.set_prod(r[0].re, u.e[0][j].re);
     im.set_prod(r[0].re, u.e[0][j].im);
-    re.sub_prod(r[0].im, u.e[0][j].im);
-    im.add_prod(r[0].im, u.e[0][j].re);
+    re.sub_prod_full(r[0].im, u.e[0][j].im);
+    im.add_prod_full(r[0].im, u.e[0][j].re);
 #pragma unroll
     for (int k = 1; k < 3; k++) {
         re.add_prod(r[k].re, u.e[k][j].re);
-        re.sub_prod(r[k].im, u.e[k][j].im);
+        re.sub_prod_full(r[k].im, u.e[k][j].im);
         im.add_prod(r[k].re, u.e[k][j].im);
-        im.add_prod(r[k].im, u.e[k][j].re);
+        im.add_prod_full(r[k].im, u.e[k][j].re);
     }
     return Cx<Df>{re.value(), im.value()};
 }
@@ -872,7 +872,7 @@ __device__ __forceinline__ double plaq_plane(const GaugeRef<PREC_DF> &U, int mu,
         unm.e[k / 3][k % 3] = df_entry(U, nu, 1 - par, k, cb_m);
         umn.e[k / 3][k % 3] = df_entry(U, mu, 1 - par, k, cb_n);
     }
-    DfAcc tr;
+    DfDot tr;
 #pragma unroll 1 // one row's code, used three times: it fits the instruction cache
     for (int i = 0; i < 3; i++) {
         Cx<Df> ru[3], rv[3];
@@ -885,7 +885,7 @@ __device__ __forceinline__ double plaq_plane(const GaugeRef<PREC_DF> &U, int mu,
         for (int j = 0; j < 3; j++) {
             const Cx<Df> a = df_row_times(ru, unm, j), b = df_row_times(rv, umn, j);
             tr.add_prod(a.re, b.re);
-            tr.add_prod(a.im, b.im);
+            tr.add_prod_full(a.im, b.im);
         }
     }
     return (double)tr.value();

@@ -26,31 +26,31 @@ __device__ __forceinline__ Df df_rsqrt(Df n)
 __device__ __forceinline__ M3<Df> reunit_rows_df(const M3<float> &e)
 {
     M3<Df> u;
-    DfAcc n0;
+    DfDot n0;
 #pragma unroll
     for (int b = 0; b < 3; b++) {
-        n0.add_prod(Df(e.e[0][b].re, 0.f), Df(e.e[0][b].re, 0.f));
-        n0.add_prod(Df(e.e[0][b].im, 0.f), Df(e.e[0][b].im, 0.f));
+        n0.add_prod_full(Df(e.e[0][b].re, 0.f), Df(e.e[0][b].re, 0.f));
+        n0.add_prod_full(Df(e.e[0][b].im, 0.f), Df(e.e[0][b].im, 0.f));
     }
     const Df s0 = df_rsqrt(n0.value());
 #pragma unroll
     for (int b = 0; b < 3; b++) u.e[0][b] = Cx<Df>{s0 * Df(e.e[0][b].re, 0.f), s0 * Df(e.e[0][b].im, 0.f)};
-    DfAcc ore, oim; // <row0, row1>
+    DfDot ore, oim; // <row0, row1>
 #pragma unroll
     for (int b = 0; b < 3; b++) {
         const Df r1(e.e[1][b].re, 0.f), i1(e.e[1][b].im, 0.f);
-        ore.add_prod(u.e[0][b].re, r1);
-        ore.add_prod(u.e[0][b].im, i1);
-        oim.add_prod(u.e[0][b].re, i1);
-        oim.sub_prod(u.e[0][b].im, r1);
+        ore.add_prod_full(u.e[0][b].re, r1);
+        ore.add_prod_full(u.e[0][b].im, i1);
+        oim.add_prod_full(u.e[0][b].re, i1);
+        oim.sub_prod_full(u.e[0][b].im, r1);
     }
     const Cx<Df> ov{ore.value(), oim.value()};
-    DfAcc n1;
+    DfDot n1;
 #pragma unroll
     for (int b = 0; b < 3; b++) {
         u.e[1][b] = Cx<Df>{Df(e.e[1][b].re, 0.f), Df(e.e[1][b].im, 0.f)} - ov * u.e[0][b];
-        n1.add_prod(u.e[1][b].re, u.e[1][b].re);
-        n1.add_prod(u.e[1][b].im, u.e[1][b].im);
+        n1.add_prod_full(u.e[1][b].re, u.e[1][b].re);
+        n1.add_prod_full(u.e[1][b].im, u.e[1][b].im);
     }
     const Df s1 = df_rsqrt(n1.value());
 #pragma unroll
@@ -100,13 +100,13 @@ __device__ __forceinline__ void link_update_one(const GaugeRef<LQCD_F64> &U, con
         for (int i = 0; i < 3; i++)
 #pragma unroll
             for (int j = 0; j < 3; j++) {
-                DfAcc re, im;
+                DfDot re, im;
 #pragma unroll
                 for (int k = 0; k < 3; k++) {
                     re.add_prod(E.e[i][k].re, u.e[k][j].re);
-                    re.sub_prod(E.e[i][k].im, u.e[k][j].im);
+                    re.sub_prod_full(E.e[i][k].im, u.e[k][j].im);
                     im.add_prod(E.e[i][k].re, u.e[k][j].im);
-                    im.add_prod(E.e[i][k].im, u.e[k][j].re);
+                    im.add_prod_full(E.e[i][k].im, u.e[k][j].re);
                 }
                 const Df vr = re.value(), vi = im.value();
                 if (write_f64) nu.e[i][j] = cx<double>((double)vr, (double)vi);
