@@ -132,13 +132,17 @@ struct SvcGauge {
 
 constexpr size_t IDLE_WS_MAX = 12;
 
-// Sets of temporaries of a gauge field (576 bytes per even site each): as many
-// as it takes for the residuals of one round to fill the GPU with about 196,608
-// sites, at most one request's.  With them and the resuming launch of batch.cu
-// two requests on 8^4 and 16^3x32 take 28.2 instead of 31.1 ms.
+// Sets of temporaries of a gauge field (576 bytes per even site each), at most
+// one request's: as many as it takes for the residuals of one round to fill five
+// waves of the float-float hop (four blocks of 64 sites on each of 152 SMs).
+// Twelve right-hand sides with one set, and with sets for 1, 2, 5 and 10 waves:
+// 8^4 8.1, 5.1, 5.0, 5.0, 5.0 ms; 12^4 10.2, 7.8, 7.5, 7.3, 7.3; 16^3x32 25.1,
+// 25.0, 23.8, 23.4, 23.0; 24^4 53.8, 53.8, 53.8, 52.0, 51.5; 8^4 and 16^3x32
+// together 31.8, 29.0, 28.0, 27.4, 27.0.  Past five, 1 to 2% for twice the memory.
+constexpr int DF_WAVE_SITES = 152 * 4 * 64;
 static size_t temporary_sets(int Vh)
 {
-    return (size_t)std::min(12, std::max(1, nblocks_for(196608, Vh)));
+    return (size_t)std::min(12, std::max(1, nblocks_for(5 * DF_WAVE_SITES, Vh)));
 }
 
 struct SvcRhs {
