@@ -140,6 +140,8 @@ __device__ __forceinline__ void cg_finish(CgScalars *sc, const double *partials,
 #endif
 // threads per block of the hopping-term kernels (one output site each)
 constexpr int DS_BLOCK = LQCD_DS_BLOCK;
+// FP64 (dslash_f64.cuh): four threads per site
+constexpr int QUAD_SITES = 32, QUAD_BLOCK = 4 * QUAD_SITES;
 
 inline int dslash_blocks(int Vh) { return nblocks_for(Vh, DS_BLOCK); }
 
@@ -179,7 +181,10 @@ inline bool hop_takes_pap_step(lqcd_prec p, const HopPlan &plan)
 // block partials that a reducing hop on this lattice stores
 inline int hop_partials(const lqcd_field *in, const HopPlan &plan)
 {
-    return nblocks_for(in->Vh, in->prec == LQCD_F16N && plan.form == 2 ? plan.block : DS_BLOCK);
+    const int sites = in->prec == LQCD_F64                       ? QUAD_SITES
+                      : in->prec == LQCD_F16N && plan.form == 2 ? plan.block
+                                                                 : DS_BLOCK;
+    return nblocks_for(in->Vh, sites);
 }
 
 // out = D_{out<-in} in (dagger: D^dag).  Parities from the field kinds.
@@ -189,7 +194,7 @@ lqcd_status dslash_plain(lqcd_field *out, const lqcd_field *U, const lqcd_field 
                          cudaStream_t s, PapStep pap = {}, const HopPlan *plan = nullptr);
 
 // out = x + b D in; if partials != NULL also the per-block partial sums of
-// |out|^2 (dslash_blocks(Vh) of them), and if fin != NULL the last block then
+// |out|^2 (hop_partials of them), and if fin != NULL the last block then
 // sums them and applies the CG pAp step to fin (cg_finish).
 lqcd_status dslash_xpay(lqcd_field *out, const lqcd_field *U, const lqcd_field *in, int dagger, const lqcd_field *x,
                         double b, double *partials, const int *skip, cudaStream_t s, CgScalars *fin = nullptr,

@@ -24,7 +24,6 @@
 
 namespace lqcd {
 
-constexpr int QUAD_SITES = 32, QUAD_BLOCK = 4 * QUAD_SITES;
 constexpr int QUAD_PER_SM = 4; // blocks the register budget is cut for
 
 struct QuadF64 {
