@@ -126,6 +126,10 @@ uint64_t lqcd_launch_count(void);
  * "gauge_force", "fermion_force", "link_update", and "dslash_f16n_plain" (the
  * plain FP16+norm hops alone, without fused epilogues; they are also counted
  * in "dslash_f16n").  Enabling clears the totals.
+ * A solve whose iterations would run in one kernel (lqcd_solver_limits) runs
+ * them kernel by kernel while its hopping-term class is timed, with the same
+ * bits: the times are those of that path's launches, which the untimed solve
+ * on such a lattice does not make.
  * lqcd_kernel_timer_read synchronises the device, then returns the summed
  * event time in milliseconds, the number of launches of one class and, for the
  * hopping-term classes, the algorithmic bytes those launches move (every

@@ -19,16 +19,17 @@
 // step and alpha in the wait behind the next hop, the update of x in the wait
 // for |r|^2, the links and neighbours of the next hop beside the epilogue.
 //
-// Measured, FP16+norm solves of about 32 iterations and 4 reliable updates,
-// kernel by kernel and resident: 4^4 1648 and 1034 us, 8^4 1835 and 1123 us,
-// 12^4 1906 and 1369 us, 16^4 2176 and 1672 us, 16^3x32 (512 blocks) 2749 and
-// 2362 us.  The overlap above, later: 8^4 941 -> 908 us, 12^4 1195 -> 1118,
-// 16^4 1484 -> 1371, 16^3x32 2160 -> 1993 (BF16 2530 -> 2398, FP32 2186 ->
-// 2067), FP64 8^4 1694 -> 1657.  Up to 16 blocks the grid is one cluster,
-// whose hardware barrier makes an iteration of 8^4 4 us shorter than the
-// barrier through L2.  The blocks have to be resident together, so the path
-// ends at 608 of them; there the kernel boundaries cost 15% and fall with the
-// number of waves, while more sites per block would leave SMs unevenly filled.
+// Measured, solves of about 30 iterations, kernel by kernel and resident:
+// FP16+norm (3 reliable updates) 4^4 924 and 762 us, 8^4 997 and 803, 12^4 1074
+// and 965, 14^4 1147 and 1022, 16^4 1351 and 1203, 16^3x32 (512 blocks) 1851 and
+// 1763; BF16 (7 updates) 8^4 1138 and 991, 16^3x32 2398 and 2307; FP32 (4) 8^4
+// 1297 and 1002, 16^3x32 2190 and 2020; FP64 8^4 1806 and 1517, 14^4 (601 blocks)
+// 4604 and 4394.  Of that the overlap above is 4% on 8^4 and 8% on 16^3x32.  Up
+// to 16 blocks the grid is one cluster, whose hardware barrier makes an
+// iteration of 8^4 4 us shorter than the barrier through L2.  The blocks have to
+// be resident together, so the path ends at 608 of them; there the kernel
+// boundaries cost 5% (FP32 8%) and fall with the number of waves, while more
+// sites per block would leave SMs unevenly filled.
 // Four threads per site on lattices of up to 152 blocks were no faster: an SM's
 // instructions are the same, and exchanging the hops adds shared-memory traffic.
 #include "cg.cuh"

@@ -9,8 +9,9 @@
 // boundary factor is applied to the half spinor of a hop across the t
 // boundary, never to the links, so 12-real compressed links stay in SU(3).
 //
-// FP64 storage uses FP64 arithmetic (four threads per site, dslash_f64.cuh); FP32, FP16+norm and BF16 storage use
-// FP32 arithmetic with 12-real links (row 2 = conj(row0 x row1)).
+// FP64 storage uses FP64 arithmetic (four threads per site, dslash_f64.cuh);
+// FP32, FP16+norm and BF16 storage use FP32 arithmetic with 12-real links
+// (row 2 = conj(row0 x row1)).
 #include <atomic>
 
 #include "df64.cuh"
@@ -25,9 +26,9 @@ namespace lqcd {
 // ---------------------------------------------------------------- kernels
 
 // Sp of D in at site cb.  FORM 1 (FP16+norm): the thread prefetches its
-// links into shared memory first; FORM 2 (FP16+norm): the same with packed
-// FP32x2 arithmetic.  FORM 0: every operand gathered by its thread.  (The
-// other precisions' FORM 1, 2 instances are never launched.)
+// links into shared memory first; FORM 2 (FP16+norm, and BF16 always): the same
+// with packed FP32x2 arithmetic.  FORM 0: every operand gathered by its thread
+// (FP32 always).
 template <typename R, lqcd_prec SP, lqcd_prec GP, bool DAG, int FORM, int BLOCK = DS_BLOCK>
 __device__ __forceinline__ Sp<R> site_value(const SpinorRef<SP> &in, const GaugeRef<GP> &U, const Geo &g, int cb,
                                             int out_par)

@@ -297,7 +297,7 @@ def set_allocator(alloc, free):
 
 def current_stream() -> int:
     """the current stream's handle.  Once PyTorch has CUDA up the handle alone
-    is asked for (0.2 us); the check for a device and a Stream object took 3.8
+    is asked for (0.3 us); the check for a device and a Stream object took 3.8
     us of a hopping term's 8 us call on 8^4"""
     import torch
 
