@@ -151,6 +151,10 @@ inline int dslash_blocks(int Vh) { return nblocks_for(Vh, DS_BLOCK); }
 // then end with their stores; with the step in its last block (cg_finish) each
 // of them waits for a fence and an atomic.  FP16+norm axpy hop on 32^3x64 about
 // 9 us shorter (77 -> 68 us), sixteen batched chains 30.4 -> 29.6 ms.
+// A step that pauses the solve (a pAp that is not positive) sets the flag that
+// this hop's other blocks read when they start: some of them may do their sites
+// and some not, and nothing reads the hop's output, since the CG-update hop
+// behind it sees the pause.
 struct PapStep {
     CgScalars *sc = nullptr; // NULL: none
     const double *partials = nullptr;
