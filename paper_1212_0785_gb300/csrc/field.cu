@@ -896,8 +896,8 @@ __device__ __forceinline__ double plaq_plane(const GaugeRef<PREC_DF> &U, int mu,
 // for the planes with t and 1 / xi0 for the spatial ones.  One thread per site
 // and plane: the six planes of a range of PB sites are six consecutive work
 // items, so they share its links through L2 and a small lattice spreads over
-// six times as many SMs: lqcd_plaquette on 8^4 186 -> 69 us, 12^4 178 -> 102,
-// 16^3x32 586 -> 382 us, on 32^3x64 (FP64 pipe: 4.7 ms) 5.55 -> 5.19 ms.
+// six times as many SMs: lqcd_plaquette on 8^4 186 -> 65 us, 12^4 178 -> 102,
+// 16^3x32 586 -> 376 us, on 32^3x64 (FP64 pipe: 4.7 ms) 5.55 -> 5.24 ms.
 // At most PLAQ_MAX_BLOCKS blocks, each taking items blockIdx.x, + gridDim.x,
 // ...: a fixed order for a lattice.
 constexpr int PB = 128;
