@@ -198,6 +198,14 @@ struct lqcd_service {
 
 namespace lqcd {
 
+// gauge field i, for the worker thread outside the lock: lqcd_service_add_gauge
+// may be growing the list
+static SvcGauge &gauge_of(lqcd_service *S, int i)
+{
+    std::lock_guard<std::mutex> lk(S->mu);
+    return *S->gauges[i];
+}
+
 // device bytes of one right-hand side's solver work space, whose float-float
 // links and temporaries are the gauge field's
 static size_t ws_bytes(const lqcd_lattice &lat, lqcd_prec sloppy) { return cg_workspace_bytes(lat, sloppy, true); }
@@ -233,7 +241,8 @@ static lqcd_status gauge_setup(lqcd_service *S, SvcGauge &g)
     if (g.ready) return LQCD_OK;
     cudaStream_t s = S->stream;
     const lqcd_lattice &lat = g.U->lat;
-    // a set-up that failed half way starts over
+    // a set-up that failed half way starts over (once its work has ended)
+    if (g.Us.f) LQCD_CUDA(cudaStreamSynchronize(s));
     for (FieldPtr *f : {&g.Us, &g.Udf, &g.bo, &g.bp, &g.to, &g.src, &g.bo_df, &g.xo_df, &g.mxe_df}) {
         if (f->f) lqcd_field_free(f->f);
         f->f = nullptr;
@@ -279,13 +288,18 @@ static void grow_sets(lqcd_service *S, SvcGauge &g)
 // sets hold nothing between the solver's steps); returns whether any was freed
 static bool drop_sets(lqcd_service *S)
 {
+    std::vector<SvcGauge *> gauges;
+    {
+        std::lock_guard<std::mutex> lk(S->mu); // (lqcd_service_add_gauge may grow the list)
+        for (auto &g : S->gauges) gauges.push_back(g.get());
+    }
     bool any = false;
-    for (auto &g : S->gauges) {
+    for (SvcGauge *g : gauges) {
         g->one_set = true;
         if (g->shared.size() < 2) continue;
         any = true;
         for (SvcRequest *r : S->running)
-            if (S->gauges[r->req.gauge] == g)
+            if (gauges[r->req.gauge] == g)
                 for (auto &h : r->rhs)
                     if (h->ws) h->ws->tmp_from = g->shared[0].get();
         g->shared.resize(1);
@@ -421,11 +435,15 @@ static lqcd_status admit_enqueue(lqcd_service *S, SvcRequest &r, SvcGauge &g)
 
 static lqcd_status admit(lqcd_service *S, SvcRequest &r)
 {
-    SvcGauge &g = *S->gauges[r.req.gauge];
+    SvcGauge &g = gauge_of(S, r.req.gauge);
     lqcd_status rc = admit_enqueue(S, r, g);
-    if (rc == LQCD_ENOMEM && drop_sets(S)) {
-        r.rhs.clear();
-        rc = admit_enqueue(S, r, g);
+    if (rc == LQCD_ENOMEM) {
+        // what was enqueued for this request ends before its buffers go back
+        LQCD_CUDA(cudaStreamSynchronize(S->stream));
+        if (drop_sets(S)) {
+            r.rhs.clear();
+            rc = admit_enqueue(S, r, g);
+        }
     }
     LQCD_TRY(rc);
     grow_sets(S, g);
@@ -516,7 +534,7 @@ static void finish_request(lqcd_service *S, SvcRequest &r, lqcd_status st)
         if (o.status == LQCD_OK && h->status != LQCD_OK) o.status = h->status;
         // the solver fields go back to the gauge field's pool (or are freed);
         // the solution halves stay until release
-        SvcGauge &g = *S->gauges[r.req.gauge];
+        SvcGauge &g = gauge_of(S, r.req.gauge);
         if (h->ws && h->ws->ready && g.idle.size() < IDLE_WS_MAX) {
             g.idle.push_back(std::move(h->ws));
             idle_added += ws_bytes(g.U->lat, S->prm.cg.sloppy);
@@ -593,6 +611,7 @@ static lqcd_status worker_step(lqcd_service *S)
     for (SvcRequest *r : admitted) {
         lqcd_status rc = admit(S, *r);
         if (rc != LQCD_OK) {
+            cudaStreamSynchronize(S->stream); // the caller may release the buffers of what was enqueued
             for (auto &h : r->rhs) {
                 h->finalized = true;
                 h->status = rc;
@@ -605,7 +624,7 @@ static lqcd_status worker_step(lqcd_service *S)
     LQCD_TRY(S->bs.step(S->prm.cg.sloppy, S->stream));
     std::vector<SvcRequest *> still;
     for (SvcRequest *r : S->running) {
-        SvcGauge &g = *S->gauges[r->req.gauge];
+        SvcGauge &g = gauge_of(S, r->req.gauge);
         bool all = true;
         for (auto &h : r->rhs) {
             if (h->finalized) continue;

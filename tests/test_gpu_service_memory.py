@@ -18,12 +18,18 @@ TOL = 1e-10
 
 
 class CappedAllocator:
-    """device memory from PyTorch's caching allocator, NULL past cap live bytes"""
+    """device memory from PyTorch's caching allocator, NULL past cap live bytes
+    and at call number fail_at"""
 
-    def __init__(self, cap=None):
+    def __init__(self, cap=None, fail_at=None):
         self.cap, self.live, self.peak, self.sizes, self.refused = cap, 0, 0, {}, 0
+        self.fail_at, self.calls = fail_at, 0
 
     def alloc(self, nbytes, stream):
+        self.calls += 1
+        if self.calls == self.fail_at:
+            self.refused += 1
+            return None
         if self.cap is not None and self.live + nbytes > self.cap:
             self.refused += 1
             return None
@@ -81,3 +87,51 @@ def test_requests_that_fit_with_fewer_sets(order, dropped):
     assert mem.refused == 0
     got, capped = run(Uh, order, cap=mem.peak - int(dropped * SET))
     assert capped.refused > 0 and same(free, got)
+
+
+def test_allocation_failure_at_every_allocation():
+    """of a first request's admission and solve: it is refused for want of memory
+    or solved with the same bits, nothing leaks, and a service that goes on
+    (a failed admission does not stop it) solves the next request"""
+    Uh = orc.gauge_start(DIMS, seed=30, eps=0.25)
+
+    def ask(svc, gid, mem):
+        t = svc.submit(gid, 0.152, (1, 2, 3, 0), 3)
+        r = svc.wait(t)
+        calls, mem.fail_at = mem.calls, None  # (the download has a buffer of its own)
+        xs = []
+        if r["status"] == lqcd.OK:
+            xs = [lqcd.Field.borrowed(h, DIMS, lqcd.SPINOR_EVEN).download() for h in
+                  (svc.solution(t, k)[0] for k in range(3))]
+        svc.release(t)
+        return r["status"], xs, calls
+
+    U = lqcd.gauge_field(DIMS).upload(Uh)
+    want, total, refused, solved, stopped, k = None, None, 0, 0, 0, 0
+    while total is None or k <= total:
+        mem = CappedAllocator(fail_at=k or None)
+        lqcd.set_allocator(mem.alloc, mem.free)
+        try:
+            svc = lqcd.Service(lqcd.service_params(tol=TOL))
+            gid = svc.add_gauge(U)
+            status, xs, calls = ask(svc, gid, mem)
+            if want is None:
+                want, total = xs, calls
+            assert status in (lqcd.OK, lqcd.ENOMEM) and (k == 0 or mem.refused == 1)
+            if status == lqcd.OK:
+                solved += 1
+                assert all(np.array_equal(a, b) for a, b in zip(xs, want))
+            else:
+                refused += 1
+                try:
+                    status, xs, _ = ask(svc, gid, mem)
+                    assert status == lqcd.OK and all(np.array_equal(a, b) for a, b in zip(xs, want))
+                except lqcd.LqcdError as e:
+                    assert e.status == lqcd.ENOMEM  # the solver's tables: the service has stopped
+                    stopped += 1
+            svc.close()
+            assert mem.live == 0, k
+        finally:
+            lqcd.set_allocator(None, None)
+        k += 1
+    assert refused > 10 and solved > 10 and stopped < 6
